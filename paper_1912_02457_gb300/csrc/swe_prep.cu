@@ -118,9 +118,8 @@ constexpr int kBathyStrip = 26, kBathyWarps = 4;
 
 template <bool INIT, bool STATS>
 __global__ void __launch_bounds__(kBathyWarps * 32) bathy_march_kernel(
-    const float *__restrict__ Hm, long long pitch, int nx, int ny, const float *__restrict__ X, long long xp,
-    float *__restrict__ Y, long long yp, float half_theta, float inv_2theta, float wgt, int rows,
-    unsigned int *misfit, unsigned int *change) {
+    const float *Hm, long long pitch, int nx, int ny, const float *X, long long xp, float *Y, long long yp,
+    float half_theta, float inv_2theta, float wgt, int rows, unsigned int *misfit, unsigned int *change) {
     constexpr unsigned full = 0xffffffffu;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int base = (blockIdx.x * kBathyWarps + warp) * kBathyStrip - 3;
@@ -128,7 +127,10 @@ __global__ void __launch_bounds__(kBathyWarps * 32) bathy_march_kernel(
     const int J0 = blockIdx.y * rows, J1 = min(J0 + rows, ny + 1);
     float mis = 0.f, chg = 0.f;
     // the next iteration's blocks may start; this one's first loads need the
-    // iteration before it
+    // iteration before it. That one, and the two before it, may still run while
+    // this block is resident, so a line of either plane that an L1 holds can be
+    // two iterations old and no plane is read-only for this kernel's lifetime:
+    // the planes are read from L2 (__ldcg), never through the non-coherent path.
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");
     if (base + 3 <= nx) {                        // (warp-uniform: the strip has a corner)
@@ -196,15 +198,15 @@ __global__ void __launch_bounds__(kBathyWarps * 32) bathy_march_kernel(
             if (inside(k0)) {
 #pragma unroll
                 for (int q = 0; q < 4; q++) {
-                    x[q] = INIT ? 0.f : __ldg(px + q * xp);
-                    h[q] = __ldg(ph + q * pitch);
+                    x[q] = INIT ? 0.f : __ldcg(px + q * xp);
+                    h[q] = __ldcg(ph + q * pitch);
                 }
             } else {
 #pragma unroll
                 for (int q = 0; q < 4; q++) {
                     const int k = k0 + q;
-                    x[q] = !INIT && corner && k >= 0 && k <= ny ? __ldg(px + q * xp) : 0.f;
-                    h[q] = cell && k >= 0 && k < ny ? __ldg(ph + q * pitch) : 0.f;
+                    x[q] = !INIT && corner && k >= 0 && k <= ny ? __ldcg(px + q * xp) : 0.f;
+                    h[q] = cell && k >= 0 && k < ny ? __ldcg(ph + q * pitch) : 0.f;
                 }
             }
             px += 4 * xp;
