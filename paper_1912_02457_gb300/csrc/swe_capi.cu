@@ -53,7 +53,8 @@ struct swe_domain {
     swe_alloc_fn alloc = nullptr;
     swe_free_fn release = nullptr;
     void *alloc_ctx = nullptr;
-    std::vector<void *> owned;
+    struct Buffer { void *ptr, *base; };   // base: as the allocator gave it
+    std::vector<Buffer> owned;
     // components of the state (two buffers), increment and Kahan terms, their
     // cells `stride` elements apart: planes (1), or one Vec4 per cell (4, the
     // fast path)
@@ -112,30 +113,41 @@ struct swe_domain {
     bool fast() const { return prec != SWE_F64 && march(); }
     int parts() const { return fast() ? swe::fast_step_parts(p.cfl_faces != 0) : swe::ref_step_parts(); }
 
-    void *dalloc(size_t bytes) {
+    void *raw_alloc(size_t bytes) {
+        if (alloc) return alloc(bytes, stream, alloc_ctx);
         void *ptr = nullptr;
-        if (alloc) {
-            ptr = alloc(bytes, stream, alloc_ctx);
-        } else if (cudaMalloc(&ptr, bytes) != cudaSuccess) {
-            ptr = nullptr;
+        return cudaMalloc(&ptr, bytes) == cudaSuccess ? ptr : nullptr;
+    }
+    void raw_free(void *base) {
+        if (release) release(base, stream, alloc_ctx);
+        else cudaFree(base);
+    }
+    // A cell's vector is read and written sixteen bytes at a time; an allocator
+    // that promises less is asked for room to round its address up.
+    void *dalloc(size_t bytes) {
+        constexpr uintptr_t kAlign = alignof(swe::Vec4<float>);
+        void *base = raw_alloc(bytes);
+        if (base && (uintptr_t)base % kAlign) {
+            raw_free(base);
+            base = raw_alloc(bytes + kAlign - 1);
         }
-        if (ptr) {
-            try {
-                owned.push_back(ptr);
-            } catch (...) {                      // no exception crosses the C ABI
-                if (release) release(ptr, stream, alloc_ctx);
-                else cudaFree(ptr);
-                ptr = nullptr;
-            }
+        if (!base) return nullptr;
+        void *ptr = (void *)(((uintptr_t)base + kAlign - 1) / kAlign * kAlign);
+        try {
+            owned.push_back({ptr, base});
+        } catch (...) {                          // no exception crosses the C ABI
+            raw_free(base);
+            ptr = nullptr;
         }
         return ptr;
     }
     void dfree(void *ptr) {
-        if (!ptr) return;
         for (size_t k = 0; k < owned.size(); k++)
-            if (owned[k] == ptr) { owned.erase(owned.begin() + (long)k); break; }
-        if (release) release(ptr, stream, alloc_ctx);
-        else cudaFree(ptr);
+            if (owned[k].ptr == ptr) {
+                raw_free(owned[k].base);
+                owned.erase(owned.begin() + (long)k);
+                break;
+            }
     }
     void free_all() {
         drop_graph();
@@ -143,10 +155,7 @@ struct swe_domain {
         capture_stream = nullptr;
         for (cudaEvent_t e : events) cudaEventDestroy(e);
         events.clear();
-        for (void *ptr : owned) {
-            if (release) release(ptr, stream, alloc_ctx);
-            else cudaFree(ptr);
-        }
+        for (const Buffer &b : owned) raw_free(b.base);
         owned.clear();
     }
     size_t plane_bytes() const { return (size_t)pitch * ny * esz; }
