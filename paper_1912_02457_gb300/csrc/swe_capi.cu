@@ -354,14 +354,28 @@ int upload_plane(swe_domain *d, void *dst, const void *src, int rows, int cols,
 // step fills are land, whose increment is discarded).
 void *staging(swe_domain *d) { return d->d1[0]; }
 
+// Can this device's kernels use a caller's device pointer as it is? Memory of
+// another device, and elements off their own boundary, take a copy instead.
+bool kernel_reach(const swe_domain *d, const void *ptr) {
+    int dev = -1;
+    cudaPointerAttributes a;
+    if ((uintptr_t)ptr % d->esz) return false;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaPointerGetAttributes(&a, ptr) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return a.type == cudaMemoryTypeManaged || (a.type == cudaMemoryTypeDevice && a.device == dev);
+}
+
 template <typename T>
 int pack_state(swe_domain *d, const swe_domain_desc *dd) {
     const void *src[4] = {dd->eta, dd->hu, dd->hv, dd->f};
     const size_t n = (size_t)d->nx * d->ny;
-    for (int k = 0; k < 4 && !dd->src_is_device; k++) {
-        if (!src[k]) continue;
+    for (int k = 0; k < 4; k++) {
+        if (!src[k] || (dd->src_is_device && kernel_reach(d, src[k]))) continue;
         T *dst = (T *)staging(d) + k * n;
-        CK(cudaMemcpyAsync(dst, src[k], n * sizeof(T), cudaMemcpyHostToDevice, d->stream));
+        CK(cudaMemcpyAsync(dst, src[k], n * sizeof(T),
+                           dd->src_is_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, d->stream));
         src[k] = dst;
     }
     CK(swe::launch_pack_state<T>((const T *)src[0], (const T *)src[1], (const T *)src[2], (const T *)src[3],
@@ -754,26 +768,30 @@ int swe_read_state(swe_handle h, int field, void *dst, int dst_is_device) {
     if (!comp && (field < SWE_ETA || field > SWE_HV)) return SWE_ERR_INVALID_ARG;
     const void *q0 = comp ? h->comp[field - SWE_COMP_ETA] : h->q[0][field];
     const void *q1 = comp ? q0 : h->q[1][field];
-    if (dst_is_device || h->march()) {
+    const size_t n = (size_t)h->nx * h->ny, row = (size_t)h->nx * h->esz;
+    const cudaMemcpyKind kind = dst_is_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
+    if (h->march() || (dst_is_device && !comp)) {
         // the current buffer is known only to the device: copy by kernel, for
-        // a host dst of the march's layout through its staging room
-        void *to = dst_is_device ? dst : staging(h);
+        // a dst of the march's layout that no kernel reaches through its
+        // staging room
+        void *to = h->march() && !(dst_is_device && kernel_reach(h, dst)) ? staging(h) : dst;
         cudaError_t e = h->prec == SWE_F64
             ? swe::launch_read_plane<double>(h->ctl, (const double *)q0, (const double *)q1, h->pitch, h->stride,
                                              h->nx, h->ny, (double *)to, h->stream)
             : swe::launch_read_plane<float>(h->ctl, (const float *)q0, (const float *)q1, h->pitch, h->stride,
                                             h->nx, h->ny, (float *)to, h->stream);
         if (e != cudaSuccess) return cuda_fail(e);
-        if (dst_is_device) return SWE_OK;
-        CK(cudaMemcpyAsync(dst, to, (size_t)h->nx * h->ny * h->esz, cudaMemcpyDeviceToHost, h->stream));
+        if (to != dst) CK(cudaMemcpyAsync(dst, to, n * h->esz, kind, h->stream));
     } else {
         int par = 0;
-        CK(cudaStreamSynchronize(h->stream));
-        CK(cudaMemcpy(&par, &h->ctl->parity, sizeof par, cudaMemcpyDeviceToHost));
-        CK(cudaMemcpy2DAsync(dst, (size_t)h->nx * h->esz, par & 1 ? q1 : q0, (size_t)h->pitch * h->esz,
-                             (size_t)h->nx * h->esz, (size_t)h->ny, cudaMemcpyDeviceToHost, h->stream));
+        if (!comp) {
+            CK(cudaStreamSynchronize(h->stream));
+            CK(cudaMemcpy(&par, &h->ctl->parity, sizeof par, cudaMemcpyDeviceToHost));
+        }
+        CK(cudaMemcpy2DAsync(dst, row, par & 1 ? q1 : q0, (size_t)h->pitch * h->esz, row, (size_t)h->ny, kind,
+                             h->stream));
     }
-    CK(cudaStreamSynchronize(h->stream));
+    if (!dst_is_device) CK(cudaStreamSynchronize(h->stream));
     return SWE_OK;
 }
 
@@ -793,8 +811,9 @@ int swe_write_state(swe_handle h, int field, const void *src, int src_is_device)
     void *d0 = comp ? h->comp[field - SWE_COMP_ETA] : h->q[0][field];
     void *d1 = comp ? nullptr : h->q[1][field], *zero = comp ? nullptr : h->comp[field];
     if (h->march()) {
-        if (!src_is_device) {
-            CK(cudaMemcpyAsync(staging(h), src, (size_t)h->nx * h->ny * h->esz, cudaMemcpyHostToDevice, h->stream));
+        if (!(src_is_device && kernel_reach(h, src))) {
+            CK(cudaMemcpyAsync(staging(h), src, (size_t)h->nx * h->ny * h->esz,
+                               src_is_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, h->stream));
             src = staging(h);
         }
         if (h->prec == SWE_F64)
