@@ -257,8 +257,8 @@ int ensure_wet(swe_domain *d) {
     unsigned char *dev = (unsigned char *)d->dalloc(n);
     if (!dev) { d->wet.clear(); return SWE_ERR_OOM; }
     cudaError_t e = d->prec == SWE_F64
-        ? swe::launch_wet_strips((const double *)d->H, d->cpitch, d->nx, d->ny, dev, d->stream)
-        : swe::launch_wet_strips((const float *)d->H, d->cpitch, d->nx, d->ny, dev, d->stream);
+        ? swe::launch_wet_strips((const double *)d->H, d->cpitch, d->nx, d->ny, dev, d->ctl, d->stream)
+        : swe::launch_wet_strips((const float *)d->H, d->cpitch, d->nx, d->ny, dev, d->ctl, d->stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(d->wet.data(), dev, n, cudaMemcpyDeviceToHost, d->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(d->stream);
     d->dfree(dev);

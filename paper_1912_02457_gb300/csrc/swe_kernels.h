@@ -60,7 +60,8 @@ void fast_plan(int nx, int ny, const unsigned char *wet, const int bc[4], int fr
                bool alone, std::vector<uint2> &items);
 int fast_tiles(int n_items);
 template <typename T>
-cudaError_t launch_wet_strips(const T *H, long long cpitch, int nx, int ny, unsigned char *out, cudaStream_t st);
+cudaError_t launch_wet_strips(const T *H, long long cpitch, int nx, int ny, unsigned char *out, StepCtl *ctl,
+                              cudaStream_t st);
 // gridded: some domain of the batch has gridded wind (the kernel with the
 // per-cell wind sampling); a single domain's launch decides by its own wind.
 cudaError_t launch_batch_stage(const BatchTable &tab, int blocks, int stage, bool gridded, cudaStream_t st);

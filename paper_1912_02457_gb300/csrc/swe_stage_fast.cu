@@ -494,12 +494,17 @@ int fast_tiles(int n_items) { return (n_items + kPairs - 1) / kPairs; }
 
 // Per 28-column strip s and row j (out[s * ny + j], strip-major for the
 // planner's walk down each strip): 0 where the strip holds no wet cell of row
-// j (a cell is land when any of its corners is LAND, as in the march), kWet,
-// plus kRough where a lane of the march holds land or bed above the reference
-// level (a drying shelf): those rows take the march's slow path.
+// j (a cell is land when any of its corners is LAND), kWet, plus kRough where a
+// lane of the march holds land or bed above the reference level (a drying
+// shelf): those rows take the march's slow path.
+//
+// The march tells land by the sum of a cell's corners, at least LAND if one of
+// them is. Depths no water has (infinite, or not a number in FP64) reach that
+// sum without being land: the march would take such a cell for a coast, where
+// the scheme gives no finite state. They are a numeric error of the domain.
 template <typename T>
 __global__ void wet_strips_kernel(const T *__restrict__ H, long long cpitch, int nx, int ny, int strips,
-                                  unsigned char *__restrict__ out) {
+                                  unsigned char *__restrict__ out, StepCtl *ctl) {
     const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (t >= (long long)ny * strips) return;
     const int j = (int)(t / strips), s = (int)(t % strips);
@@ -507,23 +512,25 @@ __global__ void wet_strips_kernel(const T *__restrict__ H, long long cpitch, int
     const T *r0 = H + (long long)j * cpitch, *r1 = r0 + cpitch;
     bool wet = false, rough = false;
     for (int i = max(c0 - 2, 0); i < min(c1 + 2, nx); i++) {
-        const T sum = r0[i] + r0[i + 1] + r1[i] + r1[i + 1];
+        const T sum = (r0[i] + r0[i + 1]) + (r1[i] + r1[i + 1]);
         const bool land = r0[i] == kLand || r0[i + 1] == kLand || r1[i] == kLand || r1[i + 1] == kLand;
         wet |= !land && i >= c0 && i < c1;
         rough |= land || sum < T(0);
+        if (!land && !(sum < T(kLand))) flag_error(ctl, j * nx + i);
     }
     out[(long long)s * ny + j] = wet ? (rough ? kWet | kRough : kWet) : 0;
 }
 
 template <typename T>
-cudaError_t launch_wet_strips(const T *H, long long cpitch, int nx, int ny, unsigned char *out, cudaStream_t st) {
+cudaError_t launch_wet_strips(const T *H, long long cpitch, int nx, int ny, unsigned char *out, StepCtl *ctl,
+                              cudaStream_t st) {
     const int strips = fast_strips(nx);
     const long long n = (long long)ny * strips;
-    wet_strips_kernel<T><<<(unsigned)((n + 255) / 256), 256, 0, st>>>(H, cpitch, nx, ny, strips, out);
+    wet_strips_kernel<T><<<(unsigned)((n + 255) / 256), 256, 0, st>>>(H, cpitch, nx, ny, strips, out, ctl);
     return cudaGetLastError();
 }
-template cudaError_t launch_wet_strips<float>(const float *, long long, int, int, unsigned char *, cudaStream_t);
-template cudaError_t launch_wet_strips<double>(const double *, long long, int, int, unsigned char *, cudaStream_t);
+template cudaError_t launch_wet_strips<float>(const float *, long long, int, int, unsigned char *, StepCtl *, cudaStream_t);
+template cudaError_t launch_wet_strips<double>(const double *, long long, int, int, unsigned char *, StepCtl *, cudaStream_t);
 
 // The external edge state of the current time level (stage-1 brackets).
 __global__ void __launch_bounds__(256) edge_fill_kernel(const StageArgs<float> a) {
