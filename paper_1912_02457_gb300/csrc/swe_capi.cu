@@ -287,7 +287,10 @@ int domain_items(swe_domain *d, int budget, bool alone, const uint2 **dev, int *
     if (rc) return rc;
     std::vector<uint2> items;
     try {
-        swe::fast_plan(d->nx, d->ny, d->wet.data(), d->bc, d->p.frs_width, budget, alone, items);
+        const bool f64 = d->prec == SWE_F64;
+        swe::fast_plan(d->nx, d->ny, d->wet.data(), d->bc, d->p.frs_width, budget,
+                       f64 ? swe::f64_pairs() : swe::fast_pairs(),
+                       !alone ? 0 : f64 ? swe::f64_resident() : swe::fast_slots(), items);
     } catch (...) {
         return SWE_ERR_OOM;
     }

@@ -54,10 +54,14 @@ enum : unsigned char { kWet = 1, kRough = 2 };   // flags of launch_wet_strips
 int fast_strips(int nx);
 int fast_slots();                        // resident items of the FP32 kernels
 int f64_slots();                         // items to aim at in FP64
+int f64_resident();                      // resident items of the FP64 kernels
+int fast_pairs();                        // items of a block, FP32 and FP64
+int f64_pairs();
 int fast_budget(int nx, int ny, const unsigned char *wet, const int bc[4], int frs_width, int slots);
-// alone: the plan of a domain launched by itself (a batch launches many)
+// per_block: items a block takes; slots: the items one wave of the kernel holds,
+// 0 for a domain of a batch (which launches many)
 void fast_plan(int nx, int ny, const unsigned char *wet, const int bc[4], int frs_width, int budget,
-               bool alone, std::vector<uint2> &items);
+               int per_block, int slots, std::vector<uint2> &items);
 int fast_tiles(int n_items);
 template <typename T>
 cudaError_t launch_wet_strips(const T *H, long long cpitch, int nx, int ny, unsigned char *out, StepCtl *ctl,

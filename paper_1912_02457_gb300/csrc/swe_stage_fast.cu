@@ -411,7 +411,7 @@ int fast_budget(int nx, int ny, const unsigned char *wet, const int bc[4], int f
 }
 
 void fast_plan(int nx, int ny, const unsigned char *wet, const int bc[4], int frs_width, int budget,
-               bool alone, std::vector<uint2> &items) {
+               int per_block, int slots, std::vector<uint2> &items) {
     items.clear();
     const PlanCtx p = plan_ctx(nx, ny, wet, bc, frs_width);
     std::vector<long long> pref, cost;
@@ -437,7 +437,7 @@ void fast_plan(int nx, int ny, const unsigned char *wet, const int bc[4], int fr
         }
     }
     if (items.empty()) { items.push_back(make_uint2(0u, 1u << 16)); cost.push_back(1); }
-    const int n = (int)items.size(), nb = (n + kPairs - 1) / kPairs;
+    const int n = (int)items.size(), nb = (n + per_block - 1) / per_block;
     const auto row_major = [&](int a, int c) {
         const unsigned ja = items[a].y & 0xffffu, jc = items[c].y & 0xffffu;
         return ja != jc ? ja < jc : items[a].x < items[c].x;
@@ -446,7 +446,7 @@ void fast_plan(int nx, int ny, const unsigned char *wet, const int bc[4], int fr
     for (int k = 0; k < n; k++) order[k] = k;
     std::vector<uint2> out;
     out.reserve(n);
-    if (!alone || n > fast_slots() || budget < 8 * kPlanUnit) {
+    if (n > slots || budget < 8 * kPlanUnit) {
         // part of a batch, several waves, or short items: row-major order,
         // a block's warps taking neighbouring strips of the same rows (they
         // share halo lines in L1, which short items and later waves depend
@@ -456,11 +456,11 @@ void fast_plan(int nx, int ny, const unsigned char *wet, const int bc[4], int fr
         items.swap(out);
         return;
     }
-    // one wave of long items: blocks of kPairs items with equal total cost
+    // one wave of long items: blocks of per_block items with equal total cost
     // (largest item first to the lightest block with room), so that the SMs,
-    // whichever blocks they get, carry equal work (coastal 1024^2: +2.6%);
-    // within a block, row-major order. (When the item count is not a
-    // multiple of kPairs a packed block other than the last may hold fewer
+    // whichever blocks they get, carry equal work (coastal 1024^2: +2.6%; FP64
+    // 512 x 384 290.6 -> 282.5 us a step in its blocks of two items); within a block, row-major order. (When the item count is not a
+    // multiple of per_block a packed block other than the last may hold fewer
     // items, and the launch's blocks then straddle packed blocks after it;
     // keeping every short block last measured no different.)
     std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return cost[a] > cost[b]; });
@@ -472,7 +472,7 @@ void fast_plan(int nx, int ny, const unsigned char *wet, const int bc[4], int fr
         Load l = heap.top();
         heap.pop();
         blk[l.second].push_back(k);
-        if ((int)blk[l.second].size() < kPairs) heap.push(Load(l.first + cost[k], l.second));
+        if ((int)blk[l.second].size() < per_block) heap.push(Load(l.first + cost[k], l.second));
     }
     for (int b = 0; b < nb; b++) {
         std::sort(blk[b].begin(), blk[b].end(), row_major);
@@ -480,6 +480,8 @@ void fast_plan(int nx, int ny, const unsigned char *wet, const int bc[4], int fr
     }
     items.swap(out);
 }
+
+int fast_pairs() { return kPairs; }
 
 int fast_step_parts(bool faces) { return faces ? 3 : 2; }
 
