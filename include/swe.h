@@ -121,7 +121,9 @@ typedef struct {
     int precision;          /* swe_precision */
     int bc[4];              /* swe_bc per edge S, N, W, E */
     const void *eta, *hu, *hv;  /* nx*ny initial state */
-    const void *H;          /* (nx+1)*(ny+1) corner depths, SWE_LAND = land */
+    const void *H;          /* (nx+1)*(ny+1) corner depths, SWE_LAND = land; a cell
+                               whose depth is not finite is reported as
+                               SWE_ERR_NUMERIC by swe_get_info */
     const void *f;          /* nx*ny Coriolis parameter, or NULL: f_const */
     const void *theta;      /* nx*ny north angle (rad), or NULL: theta_const */
     double f_const, theta_const;
@@ -214,7 +216,13 @@ int swe_step_profiled(swe_handle h, int n_steps, float *ms, int capacity);
 
 /* Copy one field of the current state (nx*ny, row-major, element type of
  * the domain's precision) to dst, host or device memory. Stream-ordered;
- * for a host dst the call synchronises the stream before returning. */
+ * for a host dst the call synchronises the stream before returning.
+ * Between host memory and the default kernels' cell vectors (and between them
+ * and device memory that this device's kernels cannot address, or not on the
+ * elements' own boundary) the field passes through the buffer of the stage-1
+ * increment, which a step fills before it reads it: like every call on a
+ * domain, not while a batch or a decomposition steps it on another stream.
+ * The same holds for swe_write_state. */
 int swe_read_state(swe_handle h, int field, void *dst, int dst_is_device);
 
 /* Overwrite one field of the current state from src (same layout). Land

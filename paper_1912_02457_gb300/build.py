@@ -97,7 +97,7 @@ def build(force: bool = False, verbose: bool = False, extra_flags=(), variant: s
 
 def build_debug(force: bool = False) -> str:
     """The bounds-checked variant (_build/debug/libswe.so): every global
-    access of the FP32 stage kernels checks its offset against the extent of
+    access of the stage kernels checks its offset against the extent of
     its buffer; a violation is skipped and reported as SWE_ERR_BOUNDS with
     the source line in swe_info.error_cell. A test tool, slower than the
     product."""

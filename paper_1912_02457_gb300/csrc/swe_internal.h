@@ -94,15 +94,15 @@ struct StageArgs {
     float frs_alpha_f[kMaxFrs];   // the same weights rounded once for FP32 kernels
     StepCtl *ctl;
     ClockParams clk;
-    // FP32 fast path: the external state of Section 3.6 and f on the two
-    // ghost rings of every nested edge, one copy per time level (two levels,
-    // selected by the step parity); NULL on the other paths. A level holds
+    // the march (FP32 and FP64): the external state of Section 3.6 and f on the
+    // two ghost rings of every nested edge, one copy per time level (two levels,
+    // selected by the step parity); NULL for the reference kernels. A level holds
     // 4 (nx + ny) entries: edge S at 0, N at 2 nx, W at 4 nx, E at
     // 4 nx + 2 ny; ring r of an edge of length n at position k: r n + k.
     Vec4<T> *edge;
-    // FP32 fast path: the warp items a launch covers, {strip, j0 | rows << 16}
-    // (rows without a wet cell in the strip are left out: land cells are
-    // never written).
+    // the march: the items a launch covers, {strip, j0 | rows << 16} (rows
+    // without a wet cell in the strip are left out: land cells are never
+    // written).
     const uint2 *items;
     int n_items;
     // elements of each buffer (checked by the bounds-checked debug builds)

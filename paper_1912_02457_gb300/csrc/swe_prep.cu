@@ -1,8 +1,9 @@
 // swe_prep.cu -- grid pre-processing of libswe (Sections 3.8 and 3.9):
 // corner bathymetry from cell averages, land erosion, refinement and
-// coarsening by two. Memory-bound stencils, one thread per output point,
-// 32-wide rows for coalesced access; the neighbours of a point come
-// through L1. Nothing here allocates.
+// coarsening by two. The corner bathymetry is a march, a warp per strip of
+// columns, bound by instruction issue; the others are memory-bound stencils, two
+// or four cells per thread with vector loads and stores where the caller's layout
+// allows them, else one. Nothing here allocates.
 #include <cuda_runtime.h>
 
 #include <cstdint>

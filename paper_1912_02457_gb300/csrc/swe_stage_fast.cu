@@ -39,7 +39,9 @@ static_assert(kStrip == kStripColumns, "the planner's strips are the march's");
 constexpr int kPairs = 4;            // items per block, two warps each
 constexpr int kThreads = kPairs * 64;
 // resident blocks per SM the register budgets target: 64 registers without a
-// spill for a single domain and for stage 1 of a batch; stage 2 of a batch,
+// spill for a single domain and for stage 1 of a batch with uniform winds (with
+// gridded ones that stage spills 8 bytes at 64 registers: a 12-domain ensemble with
+// gridded winds takes 410 us a step, at 80 registers 428); stage 2 of a batch,
 // whose arguments are in shared memory, needs 80 (at 64 it spills, and with the
 // shared memory of the rings the L1 cache left over is too small for spills:
 // 12.9 -> 22.2 ms on a 12-domain ensemble of 32 steps). Domains of a batch seldom
@@ -459,10 +461,11 @@ void fast_plan(int nx, int ny, const unsigned char *wet, const int bc[4], int fr
     // one wave of long items: blocks of per_block items with equal total cost
     // (largest item first to the lightest block with room), so that the SMs,
     // whichever blocks they get, carry equal work (coastal 1024^2: +2.6%; FP64
-    // 512 x 384 290.6 -> 282.5 us a step in its blocks of two items); within a block, row-major order. (When the item count is not a
-    // multiple of per_block a packed block other than the last may hold fewer
-    // items, and the launch's blocks then straddle packed blocks after it;
-    // keeping every short block last measured no different.)
+    // 512 x 384 290.6 -> 282.5 us a step in its blocks of two items); within a
+    // block, row-major order. (When the item count is not a multiple of per_block
+    // a packed block other than the last may hold fewer items, and the launch's
+    // blocks then straddle packed blocks after it; keeping every short block last
+    // measured no different.)
     std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return cost[a] > cost[b]; });
     typedef std::pair<long long, int> Load;
     std::priority_queue<Load, std::vector<Load>, std::greater<Load>> heap;
@@ -549,13 +552,19 @@ cudaError_t launch_edge_fill(const StageArgs<float> &a, cudaStream_t st) {
 }
 
 // Stage launches carry the programmatic-stream-serialisation attribute: a
-// stage kernel that follows another stage kernel in the stream (or in a
-// captured graph) is scheduled while that kernel drains (it triggers its
-// dependents at its start); its blocks stage their arguments and load
-// their items, which no kernel writes, and then wait in
-// griddepcontrol.wait for the previous kernel's completion and its writes
-// (back-to-back steps 2.2% faster on the coastal 1024^2 step). After any
-// other stream work a launch is ordered as usual.
+// stage kernel that follows another one in the stream (or in a captured graph) is
+// scheduled once every block of that one has triggered or ended, and waits in
+// griddepcontrol.wait for its completion and its writes (back-to-back steps 2.2%
+// faster on the coastal 1024^2 step). After any other stream work a launch is
+// ordered as usual. What makes the early start safe:
+//  * before their wait the speed pass and stage 1 read what no kernel writes:
+//    arguments and items. They may be triggered by the kernel before them at its
+//    start, as the speed pass and stage 2 do.
+//  * stage 2 reads the clock and the state before its wait. So stage 1 triggers
+//    only after its own wait (previous_kernel_done): when stage 2 starts, whatever
+//    ran before stage 1 is complete, and stage 1 writes neither of the two. A
+//    trigger of stage 1 at its start would let stage 2 read them while the stage 2
+//    of the step before still writes them.
 template <typename... Params, typename... Args>
 static cudaError_t launch_stage(void (*kernel)(Params...), int blocks, cudaStream_t st, const Args &...args) {
     // one shared-memory split for all of them: an SM changes it only when idle

@@ -131,7 +131,7 @@ def bathymetry_work_bytes(nx, ny):
 
 def bathymetry_reconstruct(Hm_ptr, pitch, nx, ny, Hc_ptr, cpitch, work_ptr, n_iter=10,
                            theta=1.3, smooth=0.125, stats=True, stream=0):
-    """Corner bathymetry from FP64 cell averages; returns, when `stats`, an
+    """Corner bathymetry from FP32 cell averages; returns, when `stats`, an
     (n_iter, 2) array of the per-iteration midpoint misfit and corner change."""
     out = np.zeros(2 * max(int(n_iter), 1), dtype=np.float64) if stats else None
     _check(load().swe_bathymetry_reconstruct(
